@@ -9,6 +9,7 @@
 // K consumed in slabs of 16 staged through shared memory.  FP64 FMA on
 // GB300 is the bound, not memory.
 #include <algorithm>
+#include <utility>
 
 #include <cooperative_groups.h>
 
@@ -127,7 +128,9 @@ __global__ void __launch_bounds__(SM_T *SM_T) dgemm_small_kernel(Dgemm g, int ti
 // eight CTAs, each holding n / 8 columns in registers.  Pivot k: the owner of
 // column k sends it and the reciprocal pivot to every CTA's shared memory, one
 // cluster barrier, every CTA updates its columns; the two buffers alternate, so
-// that barrier is the only one.  One SM alone is bound by its two FP64 multiply-adds
+// that barrier is the only one per pivot.  One more comes before the first pivot (a
+// CTA's shared memory may be written only once it has started; its arrival and its
+// wait enclose the loads of A) and one after the last.  One SM alone is bound by its two FP64 multiply-adds
 // per clock (n^3 of them) and by the division that all its threads repeated: 235 us
 // at n = 64, 121 us here, of which the reciprocals are most.
 constexpr int kInvCtas = 8, kInvThreads = 256;
@@ -141,11 +144,13 @@ __global__ void __cluster_dims__(kInvCtas, 1, 1) __launch_bounds__(kInvThreads)
   cg::cluster_group cluster = cg::this_cluster();
   const int W = (n + kInvCtas - 1) / kInvCtas, j0 = (int)cluster.block_rank() * W, w = max(0, min(W, n - j0));
   double a[kInvPer];
+  auto started = cluster.barrier_arrive();
 #pragma unroll
   for (int r = 0; r < kInvPer; ++r) {
     const int e = threadIdx.x + r * kInvThreads;
     a[r] = e < n * w ? A[(e / w) * n + j0 + e % w] : 0.0;
   }
+  cluster.barrier_wait(std::move(started));
   for (int k = 0; k < n; ++k) {
     const int buf = k & 1;
 #pragma unroll

@@ -68,3 +68,28 @@ def test_fock_at_the_edges_of_its_columns_and_ranges(g, n):
     size = np.abs(h) + np.tensordot(np.abs(v), np.abs(P), axes=([3, 2], [0, 1])) + np.tensordot(
         np.abs(v), np.abs(P), axes=([1, 2], [0, 1]))
     assert np.all(np.abs(F.cpu().numpy() - (h + J - 0.5 * K)) <= 2.0 * (2 * n * n + 16) * 2.0 ** -53 * size)
+
+
+@pytest.mark.parametrize("n", [8, 64, 127])
+def test_inverse_is_the_same_whenever_its_ctas_start(g, n):
+    """The eight CTAs of the inverse write into each other's shared memory from the first pivot
+    on.  Beside work that fills the chip, so that they start at different times, it gives
+    the bits that it gives alone: nothing in it depends on the order of their start."""
+    rng = np.random.default_rng(n)
+    a = rng.normal(size=(n, n)) / np.sqrt(n)
+    dev = lambda x: torch.as_tensor(np.ascontiguousarray(x), device="cuda")
+    S, F = dev(np.eye(n) + 0.1 * (a + a.T)), dev(a + a.T)
+    big = torch.ones(1 << 26, dtype=torch.float32, device="cuda")
+    side = torch.cuda.Stream()
+    mom = [torch.zeros(4, n, n, dtype=torch.float64, device="cuda") for _ in range(33)]
+    with g.Context(n, 9, 8, 10.0) as ctx:
+        g.gf2_tail_moments(ctx.handle, S, F, 0.3, None, mom[0])
+        torch.cuda.synchronize()
+        for m in mom[1:]:
+            with torch.cuda.stream(side):
+                for _ in range(4):
+                    big.mul_(1.0)
+            g.gf2_tail_moments(ctx.handle, S, F, 0.3, None, m)
+        torch.cuda.synchronize()
+    for m in mom[1:]:
+        assert torch.equal(m, mom[0])
