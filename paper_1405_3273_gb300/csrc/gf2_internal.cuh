@@ -136,6 +136,8 @@ struct gf2_ctx {
   const void *inner_graph_key[7] = {};
   long long inner_kernels_per_iter = 0, inner_kernels_tail = 0;
 
+  int test_lost = 0;              // gf2_test_lose_arrival
+
   // small scratch
   double *d_small = nullptr;      // Sinv, basis(7), coef(4), misc: 16 N^2
   double *d_red = nullptr;        // reduction partials
@@ -235,6 +237,11 @@ gf2_status gf2_build_moment_basis(gf2_ctx *ctx, const double *S, const double *F
 // per evaluation plus the start.
 gf2_status gf2_capture_mu_search(gf2_ctx *ctx, cudaStream_t parent, cudaStream_t body_stream, const double *S,
                                  const double *F, const double *Sig, double *G, double *P, const double *prm);
+
+// Test hook.  While on != 0, the FP64 digit kernels of ctx wait for one arrival that nothing
+// gives, at the stages of the second half of their ring: their waits run out (2 s), every
+// role gives up, the kernels return and gf2_sigma_tau's FP64 result is NaN.
+extern "C" gf2_status gf2_test_lose_arrival(gf2_ctx *ctx, int on);
 
 // ---- small device helpers ----
 __host__ __device__ inline double2 cmul(double2 a, double2 b) {

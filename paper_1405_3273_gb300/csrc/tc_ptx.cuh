@@ -95,6 +95,25 @@ __device__ __forceinline__ bool mbar_wait_long(uint64_t *bar, uint32_t parity, v
   }
 }
 
+// The same for a whole warp: its lanes go on together or give up together, so that
+// no lane is left at a warp-wide instruction whose others have gone.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, volatile int *abort) {
+  if (__all_sync(0xffffffffu, mbar_try_wait_long(bar, parity))) return true;
+  const uint64_t t0 = globaltimer();
+  for (;;) {
+    if (__all_sync(0xffffffffu, mbar_try_wait_long(bar, parity))) return true;
+    if (__any_sync(0xffffffffu, *abort != 0 || globaltimer() - t0 > kWaitLimitNs)) return false;
+  }
+}
+
+// A role that ends waits for what it has in flight (loads into shared memory, MMAs), also
+// when the CTA gives up: shared and tensor memory go to the next CTA afterwards.
+__device__ __forceinline__ void mbar_drain(uint64_t *bar, uint32_t parity) {
+  const uint64_t t0 = globaltimer();
+  while (!mbar_try_wait_long(bar, parity) && globaltimer() - t0 <= kWaitLimitNs) {
+  }
+}
+
 __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, uint64_t *bar, int c0, int c1,
                                             int c2) {
   asm volatile(
