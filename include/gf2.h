@@ -55,8 +55,15 @@ typedef enum {
 /* Arithmetic of the self-energy contraction.
  *   GF2_PREC_FP64    FP64 results: every contraction as exact products of FP64
  *                    operands cut into eight 8-bit digits, FP16 tcgen05 MMAs with
- *                    exact FP32 sums, put together in integers (error at or below
- *                    that of FP64 multiply-adds).
+ *                    exact FP32 sums, put together in integers.  A sum of K terms
+ *                    errs by at most K 2^-56 times the largest entries of its row and
+ *                    its column (an FP64 multiply-add chain: by the terms that are
+ *                    there), with the basis functions first brought to one norm by
+ *                    powers of two read off v, so that a rescaled basis (v and G
+ *                    covariant) gives the same digits.  On integrals of this kind the
+ *                    error is at or below that of multiply-adds; results far below
+ *                    their row's and column's products have the absolute error of
+ *                    those.  A non-finite entry of v or G makes what it enters NaN.
  *   GF2_PREC_BF16X3  every operand split x = x_hi + x_lo into two BF16 terms,
  *                    three products hi*hi + hi*lo + lo*hi per multiply, FP32
  *                    accumulation on the tcgen05 tensor cores, FP64 for the

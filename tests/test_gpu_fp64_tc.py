@@ -186,3 +186,65 @@ def test_a_captured_call_follows_new_integrals(g, n):
             graph.replay()
             torch.cuda.synchronize()
             check(out.cpu().numpy(), G, v, (3,))
+
+
+def graded(n, spread, kind):
+    """Powers of two for n basis functions, 2^spread apart: rising, alternating or one alone."""
+    e = {"rising": np.round(np.linspace(0, spread, n)), "alternating": spread * (np.arange(n) % 2),
+         "one": spread * (np.arange(n) == n // 2)}[kind].astype(int)
+    return np.ldexp(1.0, e - spread // 2)
+
+
+@pytest.mark.parametrize("n,spread,kind", [(5, 16, "rising"), (8, 12, "alternating"), (20, 8, "rising"), (31, 30, "one"),
+                                           (40, 16, "alternating"), (64, 12, "rising"), (70, 12, "alternating")])
+@pytest.mark.parametrize("symmetric", [False, True])
+def test_basis_functions_of_different_norm(g, n, spread, kind, symmetric):
+    """v -> d d d d v and G -> G / (d d): rows of v grow along the contracted index where columns
+    of G shrink.  Eq. Sigma is covariant, and the sum of absolute terms that the
+    tolerance is taken of scales with the result: the same tolerance as everywhere."""
+    rng = np.random.default_rng(3000 + n)
+    G, v = rng.uniform(-1.0, 1.0, (9, n, n)), rng.uniform(-1.0, 1.0, (n, n, n, n))
+    if symmetric:
+        v = v + v.transpose(1, 0, 2, 3)
+    d = graded(n, spread, kind)
+    v *= d[:, None, None, None] * d[:, None, None] * d[:, None] * d
+    G /= d[:, None] * d
+    check(run(g, G, v), G, v, (0, 3, 8) if n < 60 else (3,))
+
+
+def test_integrals_with_empty_and_tiny_diagonals(g):
+    """No scale can be read off v[i][i]: functions without any integral, and a diagonal that is
+    tiny beside the rest, leave the others as accurate as they are."""
+    n = 24
+    rng = np.random.default_rng(77)
+    G, v = rng.uniform(-1.0, 1.0, (9, n, n)), rng.uniform(-1.0, 1.0, (n, n, n, n))
+    for i in range(n):
+        v[i, i] *= 2.0 ** -60
+    for i in (3, 11):
+        v[i], v[:, i], v[:, :, i], v[..., i] = 0.0, 0.0, 0.0, 0.0
+    v *= 2.0 ** -80
+    check(run(g, G, v), G, v, range(9))
+
+
+@pytest.mark.parametrize("n,m", [(6, 20), (40, 50)])
+def test_factor_order_with_basis_functions_of_different_norm(g, n, m):
+    rng = np.random.default_rng(n)
+    G, B = rng.uniform(-1.0, 1.0, (9, n, n)), rng.uniform(-1.0, 1.0, (m, n, n))
+    d = graded(n, 14, "alternating")
+    B *= d[:, None] * d
+    G /= d[:, None] * d
+    v = np.tensordot(B, B, axes=(0, 0))
+    out = torch.empty(9, n, n, dtype=torch.float64, device="cuda")
+    with g.Context(n, 9, 8, 10.0) as ctx:
+        g.gf2_set_df_integrals(ctx.handle, dev(B))
+        g.gf2_sigma_tau_df(ctx.handle, dev(G), 0, 9, out)
+        got = out.cpu().numpy()
+    # the library sums m products of B where the oracle is given v: that v's own rounding is
+    # m 2^-53 of the sums of absolute products, in the two v of Eq. Sigma
+    aW = np.tensordot(np.abs(B), np.abs(B), axes=(0, 0))
+    W = osg.exchange_combination(v)
+    for k in (0, 4, 8):
+        ref = osg.sigma_factored(G[k], osg.gbar_from_grid(G, k), v, W)
+        size = np.abs(osg.sigma_factored(np.abs(G[k]), np.abs(osg.gbar_from_grid(G, k)), aW,
+                                         2.0 * aW + aW.transpose(2, 1, 0, 3)))
+        assert np.all(np.abs(got[k] - ref) <= (2.0 ** -47 + 4 * m * 2.0 ** -53) * size)
