@@ -1,3 +1,4 @@
+import gc
 import os
 import sys
 
@@ -11,3 +12,10 @@ if ROOT not in sys.path:
 def pytest_configure(config):
     config.addinivalue_line("markers", "gpu: needs a CUDA GPU (GB300, sm_103a)")
     config.addinivalue_line("markers", "slow: takes more than a few seconds on the CPU")
+
+
+def pytest_runtest_setup(item):
+    # device tensors of earlier tests that only a garbage collection frees must not
+    # disappear between two readings of the allocated memory
+    if "no_alloc" in item.nodeid:
+        gc.collect()
