@@ -176,7 +176,8 @@ gf2_status gf2_set_df_integrals(gf2_ctx *ctx, const double *d_B, int m);
  * 2 m N^4 + 6 m N^3 flops per time point and 3 m N^2 doubles of workspace per
  * time point (chunks of up to 1 GB, allocated by the first call), no N^4
  * intermediate; for N <= 64 on the tensor cores as GF2_PREC_FP64 of gf2_sigma_tau
- * (workspace kept until the number of functions m changes), above that in FP64
+ * (workspace kept until the number of functions m changes; a captured call follows
+ * a later gf2_set_df_integrals with the same m), above that in FP64
  * multiply-adds.  The same Sigma as gf2_sigma_tau after gf2_set_df_integrals,
  * to rounding.  Grid points k0 .. k0+count-1 of the full d_G_tau
  * [n_tau][N][N]; d_Sigma_out [count][N][N].  prec: GF2_PREC_FP64 (others give

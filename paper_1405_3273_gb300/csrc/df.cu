@@ -76,7 +76,7 @@ extern "C" gf2_status gf2_set_df_integrals(gf2_ctx *ctx, const double *d_B, int 
     GF2_CK_LAUNCH(ctx, "build_wt_kernel");
   }
   ctx->df_m = m;
-  return GF2_OK;
+  return gf2_df_integrals_changed(ctx);
 }
 
 static gf2_status sigma_df_fp64(gf2_ctx *ctx, const double *d_G, int k0, int count, double *d_out) {

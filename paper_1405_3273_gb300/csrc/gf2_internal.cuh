@@ -206,6 +206,7 @@ gf2_status gf2_pole_coefficients(gf2_ctx *ctx, const double *d_moments, double *
 gf2_status gf2_integrals_ready(gf2_ctx *ctx);
 gf2_status gf2_sigma_fp64(gf2_ctx *ctx, const double *d_G_tau, int k0, int count, double *d_out);
 gf2_status gf2_sigma_df_tc(gf2_ctx *ctx, const double *d_G, int k0, int count, double *d_out);
+gf2_status gf2_df_integrals_changed(gf2_ctx *ctx);
 void gf2_df_tc_release(gf2_ctx *ctx);
 // tau -> iw of a non-equidistant grid as a product with the weights Wt[z][k][64] (real
 // and imaginary parts of 32 frequencies per z), on the same kernels

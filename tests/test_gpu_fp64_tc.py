@@ -248,3 +248,29 @@ def test_factor_order_with_basis_functions_of_different_norm(g, n, m):
         size = np.abs(osg.sigma_factored(np.abs(G[k]), np.abs(osg.gbar_from_grid(G, k)), aW,
                                          2.0 * aW + aW.transpose(2, 1, 0, 3)))
         assert np.all(np.abs(got[k] - ref) <= (2.0 ** -47 + 4 * m * 2.0 ** -53) * size)
+
+
+@pytest.mark.parametrize("n,m", [(12, 30), (40, 50)])
+def test_a_captured_factor_order_follows_new_integrals(g, n, m):
+    """Captured with its planes ready; the factor changes, its number of functions does not.
+    The replay gives what an eager call gives, up to the order of the last atomic sums."""
+    G = dev(gi.random_symmetric_g(n, 9, seed=20))
+    rng = np.random.default_rng(21)
+    out = torch.zeros(9, n, n, dtype=torch.float64, device="cuda")
+    with g.Context(n, 9, 8, 10.0) as ctx:
+        g.gf2_set_df_integrals(ctx.handle, dev(rng.uniform(-1.0, 1.0, (m, n, n))))
+        g.gf2_sigma_tau_df(ctx.handle, G, 0, 9, out)
+        torch.cuda.synchronize()
+        graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+        with torch.cuda.graph(graph, stream=side):
+            g.gf2_set_stream(ctx.handle)
+            g.gf2_sigma_tau_df(ctx.handle, G, 0, 9, out)
+        g.gf2_set_stream(ctx.handle)
+        g.gf2_set_df_integrals(ctx.handle, dev(rng.uniform(-1.0, 1.0, (m, n, n))))
+        out.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        replayed = out.cpu().numpy()
+        g.gf2_sigma_tau_df(ctx.handle, G, 0, 9, out)
+        eager = out.cpu().numpy()
+    assert np.abs(replayed - eager).max() <= 2.0 ** -44 * np.abs(eager).max()
