@@ -73,7 +73,7 @@ struct gf2_ctx {
   double vmax16 = 0.0;          // largest |v| after its FP16 scale
   int split_terms = 0;
   bool tc_pair_sym = false;     // v[i][m][q][k] = v[q][k][i][m] to rounding: the sandwich computes half the tiles
-  bool v_in_graph = false;      // a graph replaces d_v: the FP64 planes are rebuilt by every call
+  bool v_in_graph = false;      // a graph captured before the FP64 planes existed replaces d_v: calls look at its mark
   bool tc_planes_stale = false; // N > 64: the 128-wide planes are built by the first split-precision call
 
   // grid tables (built at create)
@@ -115,7 +115,7 @@ struct gf2_ctx {
   int tc_chunk = 0;
   int tc_chunk_max = 32;           // slots per split-pipeline launch (even, 2..32; the batch tuner sets it)
   int tc_pack = 1;                // time points per 64-wide tile slot (floor(64/N) for N <= 32)
-  int *d_err = nullptr;           // device error word (timeouts in tcgen05 kernels)
+  int *d_err = nullptr;           // device error word (timeouts in tcgen05 kernels), [8]: the mark of v_in_graph
   bool defer_error_check = false; // set while a batch records this context into a CUDA graph:
                                   // the split path then skips its closing read of d_err
 

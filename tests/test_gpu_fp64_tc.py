@@ -274,3 +274,42 @@ def test_a_captured_factor_order_follows_new_integrals(g, n, m):
         g.gf2_sigma_tau_df(ctx.handle, G, 0, 9, out)
         eager = out.cpu().numpy()
     assert np.abs(replayed - eager).max() <= 2.0 ** -44 * np.abs(eager).max()
+
+
+def test_integrals_set_by_a_graph_that_precedes_the_planes(g):
+    """gf2_set_integrals captured before the first FP64 call (N > 64, where it can be): calls
+    follow its replays, and pay for new planes only after one."""
+    n, nt = 96, 9
+    G = gi.random_symmetric_g(n, nt, seed=22)
+    v1, v2 = gi.random_eri(n, seed=23), gi.random_eri(n, seed=24)
+    Gd, vd, out = dev(G), dev(v1), torch.zeros(1, n, n, dtype=torch.float64, device="cuda")
+
+    def timed(ctx):
+        ms = []
+        for _ in range(7):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            g.gf2_sigma_tau_points(ctx.handle, Gd, 3, 1, out, g.GF2_PREC_FP64)
+            b.record()
+            torch.cuda.synchronize()
+            ms.append(a.elapsed_time(b))
+        return min(ms)
+
+    with g.Context(n, nt, 8, 10.0) as ctx:
+        g.gf2_set_integrals(ctx.handle, vd)
+        torch.cuda.synchronize()
+        graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+        with torch.cuda.graph(graph, stream=side):
+            g.gf2_set_stream(ctx.handle)
+            g.gf2_set_integrals(ctx.handle, vd)
+        g.gf2_set_stream(ctx.handle)
+        for v in (v1, v2, v1):
+            vd.copy_(dev(v))
+            graph.replay()
+            g.gf2_sigma_tau_points(ctx.handle, Gd, 3, 1, out, g.GF2_PREC_FP64)
+            check(out.cpu().numpy(), G, v, (3,), k0=3)
+        after_graph = timed(ctx)
+    with g.Context(n, nt, 8, 10.0) as ctx:
+        g.gf2_set_integrals(ctx.handle, vd)
+        plain = timed(ctx)
+    assert after_graph <= 1.15 * plain, (after_graph, plain)
