@@ -359,6 +359,7 @@ extern "C" gf2_status gf2_batch_tune(gf2_batch *b, const double *const *d_G_tau,
   if (cudaMalloc(&d_out, out_elems * sizeof(double)) != cudaSuccess)
     return bfail(b, GF2_ERR_NOMEM, "gf2_batch_tune: sample buffer");
   gf2_status st = GF2_OK;
+  std::vector<bool> not_fp64(b->n, false);  // instances not compared with FP64 before make_pairs
   for (int i = 0; i < b->n && st == GF2_OK; ++i) {
     const int count = std::min(32, b->n_tau[i]);
     gf2_ctx *c = b->ctx[i];
@@ -371,13 +372,17 @@ extern "C" gf2_status gf2_batch_tune(gf2_batch *b, const double *const *d_G_tau,
       cands.push_back({prec, 16});
     }
     // An instance that may share its 64-wide tiles (make_pairs) is not compared with
-    // FP64: one split build serves both systems, and FP64 on the tensor cores would
+    // FP64 yet: one split build serves both systems, and FP64 on the tensor cores would
     // win only against an unshared one and only up to N of about 40 (per point: split
     // 52 us at any N from 33 to 64; FP64 27, 49, 90 and 255 us at N = 33, 40, 48 and 64,
-    // 36, 66, 118 and 329 where v[i][m] and v[m][i] differ).
+    // 36, 66, 118 and 329 where v[i][m] and v[m][i] differ).  If no partner is left for
+    // it, it is compared afterwards.
     bool shares = false;
     for (int j = 0; j < b->n; ++j) shares = shares || can_share(b, prec, i, j);
-    if (shares && cands.size() > 1) cands.erase(cands.begin());
+    if (shares && cands.size() > 1) {
+      cands.erase(cands.begin());
+      not_fp64[i] = true;
+    }
     double best = 0.0;
     for (size_t k = 0; k < cands.size() && st == GF2_OK; ++k) {
       const Cand cd = cands[k];
@@ -409,9 +414,25 @@ extern "C" gf2_status gf2_batch_tune(gf2_batch *b, const double *const *d_G_tau,
       st = from_ctx(b, i, gf2_sigma_tau_points(c, d_G_tau[i], 0, std::min(b->n_tau[i], 2), d_out, b->path[i]));
     }
   }
+  if (st == GF2_OK) st = make_pairs(b, d_G_tau, prec);
+  for (int i = 0; i < b->n && st == GF2_OK; ++i) {
+    if (!not_fp64[i] || b->pair_of[i] >= 0) continue;
+    const int count = std::min(32, b->n_tau[i]);
+    double ms = 0.0;
+    if ((st = time_path(b, i, d_G_tau[i], d_out, 0, count, GF2_PREC_FP64, &ms)) != GF2_OK) break;
+    if (cudaStreamSynchronize(b->origin) != cudaSuccess) st = bfail(b, GF2_ERR_CUDA, "autotuner: sync");
+    const double full = ms * b->n_tau[i] / count;
+    if (full < b->est_ms[i]) {
+      gf2_tc_release(b->ctx[i]);
+      b->path[i] = GF2_PREC_FP64;
+      b->chunk[i] = 32;
+      b->est_ms[i] = full;
+    } else {
+      gf2_f64_release(b->ctx[i]);
+    }
+  }
   cudaFree(d_out);
   if (st != GF2_OK) return st;
-  if ((st = make_pairs(b, d_G_tau, prec)) != GF2_OK) return st;
   // longest estimated time first, each to the least-loaded lane
   std::vector<int> order(b->n);
   std::iota(order.begin(), order.end(), 0);

@@ -188,3 +188,45 @@ def test_shared_tiles_with_overlaps_match_oracle(g):
             assert rel <= TOL[2], i
     finally:
         b.close()
+
+
+def test_an_instance_left_without_a_partner_is_compared_with_fp64(g):
+    """34, 33 and 20 in BF16x6: one of the larger two shares tiles with the 20, the other one
+    finds no partner.  Alone it takes the path that is faster on its own (FP64 at these
+    sizes by a factor of 1.4, timed here), as an instance that never could share does."""
+    sizes, n_tau = [34, 33, 20], 65
+    Gs = [dev(gi.random_symmetric_g(n, n_tau, seed=800 + n) * 0.3) for n in sizes]
+    vs = [dev(gi.random_eri(n, seed=900 + n)) for n in sizes]
+    outs = [torch.zeros_like(x) for x in Gs]
+
+    def timed(n, v, G, out, prec):
+        with g.Context(n, n_tau, 8, 1.0) as ctx:
+            g.gf2_set_integrals(ctx.handle, v)
+            ms = []
+            for _ in range(5):
+                a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                a.record()
+                g.gf2_sigma_tau(ctx.handle, G, out, prec)
+                b.record()
+                torch.cuda.synchronize()
+                ms.append(a.elapsed_time(b))
+            return min(ms)
+
+    b = g.Batch(sizes, [n_tau] * 3)
+    try:
+        for i, v in enumerate(vs):
+            g.gf2_batch_set_system(b.handle, i, v)
+        g.gf2_sigma_tau_batched(b.handle, Gs, outs, 2)
+        partners = [g.gf2_batch_partner(b.handle, i) for i in range(3)]
+        alone = partners.index(-1)
+        assert alone in (0, 1) and partners[2] == 1 - alone
+        t = {p: timed(sizes[alone], vs[alone], Gs[alone], torch.zeros_like(Gs[alone]), p) for p in (0, 2)}
+        print("alone:", sizes[alone], "FP64", t[0], "BF16x6", t[2], "ms; plan", g.gf2_batch_plan(b.handle, alone))
+        assert t[0] < 0.9 * t[2]  # what the case rests on
+        assert g.gf2_batch_plan(b.handle, alone)[0] == 0
+        for i in range(3):
+            ref = osg.sigma_tau(Gs[i].cpu().numpy(), vs[i].cpu().numpy())
+            rel = np.abs(outs[i].cpu().numpy() - ref).max() / np.abs(ref).max()
+            assert rel <= TOL[g.gf2_batch_plan(b.handle, i)[0]], i
+    finally:
+        b.close()
