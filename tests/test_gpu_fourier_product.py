@@ -89,3 +89,19 @@ def test_large_frequency_count_takes_the_ffts(g):
             g.gf2_fft_tau_to_iw(ctx.handle, dev(X), o)
             outs.append(o.cpu().numpy()[:300])
     assert np.abs(outs[0] - outs[1]).max() <= 2.0 ** -44 * np.abs(outs[0]).max()
+
+
+@pytest.mark.parametrize("p,u", [(11, 2), (9, 8), (7, 32), (12, 1)])
+def test_end_nodes_of_steep_meshes_keep_their_digits(g, p, u):
+    """Single samples at the ends, where the intervals are up to 2^11 times shorter than in the
+    middle: X(i w_n) is that node's weight.  It is made of at most three intervals of
+    similar length with w h < 1, so neither the oracle's sum nor the library's cancels:
+    a few dozen roundings, 2^-47 of its size, cover both."""
+    M, idx = grids.power_mesh(p, u)
+    beta, n_iw, n, nt = 100.0, 8, 2, len(idx)
+    X = np.zeros((nt, n * n))
+    X[0, 0], X[-1, 1], X[1, 2], X[-2, 3] = 1.0, -1.0, 3.0, 1e-9
+    X = X.reshape(nt, n, n)
+    ref = ot.tau_to_iw_grid(X, beta, M, idx, n_iw)
+    got, _ = both_paths(g, n, M, idx, n_iw, beta, X)
+    assert np.all(np.abs(got - ref) <= 2.0 ** -47 * np.abs(ref))
