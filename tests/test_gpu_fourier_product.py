@@ -105,3 +105,28 @@ def test_end_nodes_of_steep_meshes_keep_their_digits(g, p, u):
     ref = ot.tau_to_iw_grid(X, beta, M, idx, n_iw)
     got, _ = both_paths(g, n, M, idx, n_iw, beta, X)
     assert np.all(np.abs(got - ref) <= 2.0 ** -47 * np.abs(ref))
+
+
+def test_first_call_beside_a_capture_on_another_stream(g):
+    """The first call of a context builds its planes also while another stream is under capture
+    in the strictest mode, and leaves that capture alone."""
+    M, idx = grids.power_mesh(3, 8)
+    X = np.random.default_rng(7).uniform(-1.0, 1.0, (len(idx), 3, 3))
+    Xd, out = dev(X), torch.zeros(50, 3, 3, dtype=torch.complex128, device="cuda")
+    y, own, side = torch.zeros(4, device="cuda"), torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(own):
+        ctx = g.Context(3, None, 50, 10.0, grid=(M, idx))
+    with ctx:
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=side, capture_error_mode="global"):
+            y.add_(1.0)
+            g.gf2_fft_tau_to_iw(ctx.handle, Xd, out)  # on the context's stream, not captured
+            y.add_(1.0)
+        torch.cuda.synchronize()
+        first = out.cpu().numpy()
+        graph.replay()
+        g.gf2_fft_tau_to_iw(ctx.handle, Xd, out)
+        torch.cuda.synchronize()
+    assert np.array_equal(first, out.cpu().numpy()) and float(y[0]) == 2.0
+    assert np.abs(first - ot.tau_to_iw_grid(X, 10.0, M, idx, 50)).max() <= 2.0 ** -44 * np.abs(first).max()
