@@ -146,7 +146,8 @@ gf2_status gf2_set_overlap(gf2_ctx *ctx, const double *d_S);
  * stream-ordered (its result is NaN if a bounded wait gave up).  Its workspace is
  * allocated by the first call: for N <= 64 up to 2 GB of intermediates (fewer time
  * points at a time where memory is short) and up to (128 + N) N^3 doubles of planes,
- * above that (256 + 3 N) N^3 doubles.  gf2_set_integrals rebuilds those planes once they exist, so a
+ * above that (256 + 3 N) N^3 doubles, 3 N^4 where memory is short (the planes of W then
+ * pass through in parts, N = 128 12.5 -> 19.7 ms per point).  gf2_set_integrals rebuilds those planes once they exist, so a
  * captured call follows it.  Where v_ijkl = v_jikl to the last bit, two of the four
  * FP64 contractions for N <= 64 run over the pairs j <= i.  When v has the pair symmetry (ij|kl) = (kl|ij) (checked at
  * gf2_set_integrals, to 1e-12 relative) the 64-wide path computes half of the

@@ -137,6 +137,7 @@ struct gf2_ctx {
   long long inner_kernels_per_iter = 0, inner_kernels_tail = 0;
 
   int test_lost = 0;              // gf2_test_lose_arrival
+  int test_wide_blocks = 0;       // gf2_test_wide_blocks
 
   // small scratch
   double *d_small = nullptr;      // Sinv, basis(7), coef(4), misc: 16 N^2
@@ -243,6 +244,9 @@ gf2_status gf2_capture_mu_search(gf2_ctx *ctx, cudaStream_t parent, cudaStream_t
 // gives, at the stages of the second half of their ring: their waits run out (2 s), every
 // role gives up, the kernels return and gf2_sigma_tau's FP64 result is NaN.
 extern "C" gf2_status gf2_test_lose_arrival(gf2_ctx *ctx, int on);
+// Test hook.  At N > 64 the next FP64 workspace holds at most `blocks` blocks of 256 (p, l, n)
+// of the planes of W, as where memory is short (0: all of them).
+extern "C" gf2_status gf2_test_wide_blocks(gf2_ctx *ctx, int blocks);
 
 // ---- small device helpers ----
 __host__ __device__ inline double2 cmul(double2 a, double2 b) {

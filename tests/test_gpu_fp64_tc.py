@@ -313,3 +313,22 @@ def test_integrals_set_by_a_graph_that_precedes_the_planes(g):
         g.gf2_set_integrals(ctx.handle, vd)
         plain = timed(ctx)
     assert after_graph <= 1.15 * plain, (after_graph, plain)
+
+
+@pytest.mark.parametrize("n,blocks", [(65, 33), (66, 1123), (100, 1000)])
+def test_planes_of_w_a_part_at_a_time(g, n, blocks):
+    """N > 64 where memory is short: the last stage in parts of `blocks` blocks of 256, the last
+    part smaller or a single block, and again after new integrals."""
+    import ctypes
+    f = g.lib().gf2_test_wide_blocks
+    f.argtypes, f.restype = [ctypes.c_void_p, ctypes.c_int], ctypes.c_int
+    G = gi.random_symmetric_g(n, 9, seed=25)
+    out = torch.empty(2, n, n, dtype=torch.float64, device="cuda")
+    with g.Context(n, 9, 8, 10.0) as ctx:
+        assert f(ctx.handle, blocks) == 0
+        for seed in (26, 27):
+            v = gi.random_eri(n, seed=seed)
+            g.gf2_set_integrals(ctx.handle, dev(v))
+            g.gf2_sigma_tau_points(ctx.handle, dev(G), 3, 2, out, g.GF2_PREC_FP64)
+            check(out.cpu().numpy(), G, v, (3, 4), k0=3)
+    assert f(None, 1) == 1
