@@ -93,3 +93,29 @@ def test_inverse_is_the_same_whenever_its_ctas_start(g, n):
         torch.cuda.synchronize()
     for m in mom[1:]:
         assert torch.equal(m, mom[0])
+
+
+@pytest.mark.parametrize("n", [1, 2, 10, 11, 15, 16, 22, 23, 33, 34, 35, 36, 47, 48, 52, 53, 65, 66, 71, 72, 92, 93, 100,
+                               101, 128])
+def test_dyson_at_the_edges_of_its_layouts(g, n):
+    """Either side of every size at which dyson_kernel changes its threads or elements per
+    thread, with and without Sigma.  A = (i w + mu) S - F - Sigma has an imaginary part that is
+    definite, so elimination without pivoting grows by at most a few: it errs by
+    16 n 2^-53 of |A^-1| |A| |A^-1| on either side."""
+    rng = np.random.default_rng(400 + n)
+    a = rng.normal(size=(n, n)) / np.sqrt(n)
+    S, beta, n_iw, mu = np.eye(n) + 0.1 * (a + a.T), 10.0, 5, 0.2
+    F = rng.normal(size=(n, n)) / np.sqrt(n)
+    F = F + F.T
+    w = (2 * np.arange(n_iw) + 1) * np.pi / beta
+    sig = rng.normal(size=(n_iw, n, n)) / np.sqrt(n)
+    sig = 0.1 * (sig + sig.transpose(0, 2, 1)) - 0.05j * S / w[:, None, None]
+    dev = lambda x: torch.as_tensor(np.ascontiguousarray(x), device="cuda")
+    G = torch.empty(n_iw, n, n, dtype=torch.complex128, device="cuda")
+    with g.Context(n, 9, n_iw, beta) as ctx:
+        for X in (None, sig):
+            g.gf2_dyson(ctx.handle, mu, dev(S), dev(F), None if X is None else dev(X), G)
+            A = (1j * w[:, None, None] + mu) * S - F - (0.0 if X is None else X)
+            ref = np.linalg.inv(A)
+            bound = 2 * 16 * n * 2.0 ** -53 * (np.abs(ref) @ np.abs(A) @ np.abs(ref)).max()
+            assert np.abs(G.cpu().numpy() - ref).max() <= bound
