@@ -58,12 +58,14 @@ typedef enum {
  *                    exact FP32 sums, put together in integers.  A sum of K terms
  *                    errs by at most K 2^-56 times the largest entries of its row and
  *                    its column (an FP64 multiply-add chain: by the terms that are
- *                    there), with the basis functions first brought to one norm by
- *                    powers of two read off v, so that a rescaled basis (v and G
- *                    covariant) gives the same digits.  On integrals of this kind the
- *                    error is at or below that of multiply-adds; results far below
- *                    their row's and column's products have the absolute error of
- *                    those.  A non-finite entry of v or G makes what it enters NaN.
+ *                    there).  Basis functions whose largest integrals are more than a
+ *                    factor of four apart are first brought to one norm by powers of
+ *                    two read off v, so that a rescaled basis (v and G covariant)
+ *                    keeps its digits.  For integrals of normalised functions the
+ *                    error is below that of multiply-adds relative to
+ *                    the largest entry of Sigma; an entry far below the largest (two
+ *                    distant atoms) has the absolute error of the largest, 1e-16 of it.
+ *                    A non-finite entry of v or G makes what it enters NaN.
  *   GF2_PREC_BF16X3  every operand split x = x_hi + x_lo into two BF16 terms,
  *                    three products hi*hi + hi*lo + lo*hi per multiply, FP32
  *                    accumulation on the tcgen05 tensor cores, FP64 for the
@@ -179,7 +181,8 @@ gf2_status gf2_set_df_integrals(gf2_ctx *ctx, const double *d_B, int m);
  * intermediate; for N <= 64 on the tensor cores as GF2_PREC_FP64 of gf2_sigma_tau
  * (workspace kept until the number of functions m changes; a captured call follows
  * a later gf2_set_df_integrals with the same m), above that in FP64
- * multiply-adds.  The same Sigma as gf2_sigma_tau after gf2_set_df_integrals,
+ * multiply-adds, where gf2_sigma_tau in FP64 on the same fitted integrals is the
+ * faster way (N = 128, m = 384: 12 ms per point; 2 m N^4 flops alone take 165).  The same Sigma as gf2_sigma_tau after gf2_set_df_integrals,
  * to rounding.  Grid points k0 .. k0+count-1 of the full d_G_tau
  * [n_tau][N][N]; d_Sigma_out [count][N][N].  prec: GF2_PREC_FP64 (others give
  * GF2_ERR_UNSUPPORTED).  GF2_ERR_ARG without gf2_set_df_integrals, for a NULL
@@ -201,7 +204,7 @@ gf2_status gf2_tail_moments(gf2_ctx *ctx, const double *d_S, const double *d_F, 
  *   X(tau_k) = (2/beta) sum_{n<n_iw} Re[e^{-i w_n tau_k} (X - T)(i w_n)] + T(tau_k),
  * T = the moment series of d_moments [4][N][N] resummed about a real pole
  * a = 1 hartree, T(z) = sum_r c_r (z - a)^-r, whose tau image is closed form.
- * Evaluated by one M-point FFT per matrix element (n_iw may exceed M; the
+ * Evaluated by one M/2-point FFT per matrix element (n_iw may exceed M; the
  * frequencies are folded modulo M) and written at the context's n_tau grid
  * points.  d_X_iw [n_iw][N][N] c128 in, d_X_tau [n_tau][N][N] out. */
 gf2_status gf2_fft_iw_to_tau(gf2_ctx *ctx, const double *d_X_iw, const double *d_moments,
@@ -211,13 +214,13 @@ gf2_status gf2_fft_iw_to_tau(gf2_ctx *ctx, const double *d_X_iw, const double *d
  *   X(i w_n) = int_0^beta e^{i w_n tau} X~(tau) dtau,
  * X~ = the piecewise-cubic interpolant of the samples (on [tau_a, tau_a+1]
  * the cubic through nodes a-1..a+2; nodes 0..3 and K-3..K at the ends,
- * K = n_tau - 1), integrated exactly.  Uniform grid: an M-point FFT times an
+ * K = n_tau - 1), integrated exactly.  Uniform grid: an M/2-point FFT times an
  * attenuation factor plus end-point corrections.  Non-equidistant grid
  * (gf2_create_grid): each grid interval's cubic re-expanded on the uniform
  * steps inside it, then two M-point FFTs of those coefficients (four real
- * sequences) weighted by the exact monomial integrals of one step; where
- * n_tau n_iw is small against M log2 M (up to 90 times it, and 32 n_tau n_iw bytes
- * within 1 GB), as one product with the n_tau x n_iw matrix of the integrals in the
+ * sequences) weighted by the exact monomial integrals of one step; where that is the
+ * faster way (many elements, long grids, or short grids with many frequencies; within
+ * 32 n_tau n_iw = 2^30 bytes), as one product with the n_tau x n_iw matrix of the integrals in the
  * exact digits of GF2_PREC_FP64, whose planes the first call outside a stream
  * capture builds (the FFTs until then, and where there is no room for them).
  * d_X_tau [n_tau][N][N] in, d_X_iw [n_iw][N][N] c128 out.  If d_sig12 is not NULL it receives [2][N][N] = (Sig1, Sig2), the

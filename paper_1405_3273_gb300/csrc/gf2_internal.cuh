@@ -138,6 +138,7 @@ struct gf2_ctx {
 
   int test_lost = 0;              // gf2_test_lose_arrival
   int test_wide_blocks = 0;       // gf2_test_wide_blocks
+  int test_fourier = 0;           // gf2_test_fourier_path
 
   // small scratch
   double *d_small = nullptr;      // Sinv, basis(7), coef(4), misc: 16 N^2
@@ -247,6 +248,9 @@ extern "C" gf2_status gf2_test_lose_arrival(gf2_ctx *ctx, int on);
 // Test hook.  At N > 64 the next FP64 workspace holds at most `blocks` blocks of 256 (p, l, n)
 // of the planes of W, as where memory is short (0: all of them).
 extern "C" gf2_status gf2_test_wide_blocks(gf2_ctx *ctx, int blocks);
+// Test hook.  tau -> iw on a non-equidistant grid takes the digit product (1) or the FFTs (2)
+// whatever the sizes, or the one its rule picks (0).
+extern "C" gf2_status gf2_test_fourier_path(gf2_ctx *ctx, int path);
 
 // ---- small device helpers ----
 __host__ __device__ inline double2 cmul(double2 a, double2 b) {

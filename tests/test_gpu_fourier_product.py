@@ -110,7 +110,7 @@ def test_end_nodes_of_steep_meshes_keep_their_digits(g, p, u):
 def test_first_call_beside_a_capture_on_another_stream(g):
     """The first call of a context builds its planes also while another stream is under capture
     in the strictest mode, and leaves that capture alone."""
-    M, idx = grids.power_mesh(3, 8)
+    M, idx = grids.power_mesh(11, 2)
     X = np.random.default_rng(7).uniform(-1.0, 1.0, (len(idx), 3, 3))
     Xd, out = dev(X), torch.zeros(50, 3, 3, dtype=torch.complex128, device="cuda")
     y, own, side = torch.zeros(4, device="cuda"), torch.cuda.Stream(), torch.cuda.Stream()
@@ -130,3 +130,52 @@ def test_first_call_beside_a_capture_on_another_stream(g):
         torch.cuda.synchronize()
     assert np.array_equal(first, out.cpu().numpy()) and float(y[0]) == 2.0
     assert np.abs(first - ot.tau_to_iw_grid(X, 10.0, M, idx, 50)).max() <= 2.0 ** -44 * np.abs(first).max()
+
+
+def test_the_rule_takes_the_faster_way(g):
+    """Few elements on a short grid go through the FFTs, short meshes with many frequencies and
+    long ones through the product; the slower way takes at least 1.3 times as long."""
+    import ctypes
+    f = g.lib().gf2_test_fourier_path
+    f.argtypes, f.restype = [ctypes.c_void_p, ctypes.c_int], ctypes.c_int
+    for n, (p, u), n_iw, product in ((10, (2, 64), 256, False), (4, (3, 8), 64, False), (32, (3, 8), 8192, True),
+                                     (4, (7, 32), 256, True), (64, (2, 64), 2048, True)):
+        M, idx = grids.power_mesh(p, u)
+        X = torch.randn(len(idx), n, n, dtype=torch.float64, device="cuda")
+        out = torch.empty(n_iw, n, n, dtype=torch.complex128, device="cuda")
+        us = []
+        with g.Context(n, None, n_iw, 40.0, grid=(M, idx)) as ctx:
+            for path in (0, 1, 2):
+                assert f(ctx.handle, path) == 0
+                best = []
+                for _ in range(9):
+                    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                    a.record()
+                    for _ in range(8):
+                        g.gf2_fft_tau_to_iw(ctx.handle, X, out)
+                    b.record()
+                    torch.cuda.synchronize()
+                    best.append(a.elapsed_time(b) / 8e-3)
+                us.append(min(best))
+        print(n, M, len(idx), n_iw, "rule %.1f product %.1f FFTs %.1f us" % tuple(us))
+        fast, slow = (us[1], us[2]) if product else (us[2], us[1])
+        assert slow > 1.3 * fast and us[0] < 1.15 * fast, us
+
+
+@pytest.mark.parametrize("n,p,u,n_iw", [(1, 2, 2, 1), (5, 2, 2, 31), (12, 3, 8, 32), (13, 3, 8, 33), (4, 7, 16, 300),
+                                        (4, 3, 32, 64), (3, 7, 32, 1000), (11, 3, 2, 65), (2, 2, 64, 97)])
+def test_product_at_the_edges_of_its_tiles(g, n, p, u, n_iw):
+    """As test_product_and_ffts_match_oracle, by the product whatever the rule would take."""
+    import ctypes
+    f = g.lib().gf2_test_fourier_path
+    f.argtypes, f.restype = [ctypes.c_void_p, ctypes.c_int], ctypes.c_int
+    M, idx = grids.power_mesh(p, u)
+    X = np.random.default_rng(n * 1000 + n_iw + 1).uniform(-1.0, 1.0, (len(idx), n, n))
+    out = torch.zeros(n_iw, n, n, dtype=torch.complex128, device="cuda")
+    with g.Context(n, None, n_iw, 40.0, grid=(M, idx)) as ctx:
+        assert f(ctx.handle, 1) == 0
+        g.gf2_fft_tau_to_iw(ctx.handle, dev(X), out)
+        got = out.cpu().numpy()
+    ref = ot.tau_to_iw_grid(X, 40.0, M, idx, n_iw)
+    size = ot.tau_to_iw_grid(np.abs(X), 40.0, M, idx, 1)
+    assert np.abs(got - ref).max() <= 2.0 ** -44 * 2.0 * np.abs(size[0]).max()
