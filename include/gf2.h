@@ -333,8 +333,8 @@ gf2_status gf2_natural_occupations(gf2_ctx *ctx, const double *d_P, double *d_oc
  *   gf2_batch_set_system: integrals v [N^4] of an instance (copied) and its
  *     overlap S [N][N] (may be NULL: no orthogonalisation, as gf2_set_overlap).
  *   gf2_batch_tune: autotuner.  For every instance it times each admissible
- *     path on a sample of d_G_tau[i] -- FP64 (32 points; not for an
- *     instance that may share its tiles with another one), and for N <= 64 the split tensor-core pipeline in `prec` with
+ *     path on a sample of d_G_tau[i] -- FP64 (32 points; for an instance that
+ *     may share its tiles, once it has no partner), and for N <= 64 the split tensor-core pipeline in `prec` with
  *     32 or 16 time-point slots per launch (one chunk each) -- keeps the
  *     fastest (FP64 is always admissible, being more accurate), and
  *     spreads the instances over the worker streams, longest estimated time
